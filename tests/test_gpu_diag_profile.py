@@ -82,3 +82,12 @@ def test_near_tie(B, small):
     I[32, 32] = 2.0 ** 38
     got = _diag(B, I, (-32.5, 32.5, -32.5, 32.5))
     assert got[9] == (np.floor(np.hypot(32, 32)) + 0.5 if small > 0 else 0.5)
+
+
+@pytest.mark.parametrize("half", [1e-150, 1e-30, 1e-22, 0.99e-12, 1e-12, 1e12, 1.01e12, 1e20, 1e150])
+def test_screen_scale(B, half):
+    """The peak's bin does not depend on the unit of the screen."""
+    I = np.random.default_rng(3).random((128, 128)).astype(np.float32)
+    one = _diag(B, I, (-1.0, 1.0, -1.0, 1.0))
+    got = _diag(B, I, (-half, half, -half, half))
+    assert round(got[9] / (2.0 * half / 128) - 0.5) == round(one[9] / (2.0 / 128) - 0.5)
