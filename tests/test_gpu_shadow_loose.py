@@ -33,3 +33,25 @@ def test_brackets_are_ordered(B, metric, chi, incl, rtol, lanes):
     ok = (fl & 3) == 0
     assert np.all(b_in[ok] <= b_out[ok])
     assert np.all((b_out - b_in)[ok] <= 1e-6)
+
+
+@pytest.mark.parametrize("metric,chi,incl", [(0, 0.9, 60.0), (1, 0.5, 17.0), (2, 0.95, 85.0)])
+@pytest.mark.parametrize("lanes", [0, 1, 4])
+def test_ends_have_their_fates(B, metric, chi, incl, lanes):
+    """At rtol 1e-4 the bracket is that of the FP64 integrator: the rays at its ends,
+    traced as FP64 points, are captured and not captured.  The kernels' roundings
+    differ, so a few ends next to a fold of the fates may fall on its other side:
+    one in twenty."""
+    psi = np.sort(np.random.default_rng(1).uniform(0, 2 * math.pi, 400))
+    st = B.Spacetime(metric=metric, chi=chi, lambda_E=0.3)
+    cam = B.Camera(incl=math.radians(incl))
+    it = B.Integrator(rtol=1e-4, atol=1e-6)
+    b_in, b_out, fl = (x.cpu().numpy() for x in
+                       B.shadow_boundary(st, cam, it, psi, 1.0, 9.0, 1e-9, lanes=lanes))
+    assert np.all(fl == 0)
+    wrong = 0
+    for b, captured in ((b_in, True), (b_out, False)):
+        xy = np.stack([b * np.cos(psi), b * np.sin(psi)], 1)
+        r = B.trace_points(st, cam, B.Emission(), it, xy)
+        wrong += int(np.sum((np.asarray(r["status"]) == 1) != captured))
+    assert wrong <= 40
