@@ -39,9 +39,12 @@ def test_brackets_are_ordered(B, metric, chi, incl, rtol, lanes):
 @pytest.mark.parametrize("lanes", [0, 1, 4])
 def test_ends_have_their_fates(B, metric, chi, incl, lanes):
     """At rtol 1e-4 the bracket is that of the FP64 integrator: the rays at its ends,
-    traced as FP64 points, are captured and not captured.  The kernels' roundings
-    differ, so a few ends next to a fold of the fates may fall on its other side:
-    one in twenty."""
+    traced as FP64 points (each 28 times over: enough points for the kernel that
+    gives a ray one thread, as the shadow's; the four-lane kernel of fewer points
+    rounds in another order, which at this tolerance moves the transition by more
+    than the bracket), are captured and not captured.  The two builds may still
+    round apart, so a few ends next to a fold of the fates may fall on its other
+    side: one in twenty."""
     psi = np.sort(np.random.default_rng(1).uniform(0, 2 * math.pi, 400))
     st = B.Spacetime(metric=metric, chi=chi, lambda_E=0.3)
     cam = B.Camera(incl=math.radians(incl))
@@ -51,7 +54,7 @@ def test_ends_have_their_fates(B, metric, chi, incl, lanes):
     assert np.all(fl == 0)
     wrong = 0
     for b, captured in ((b_in, True), (b_out, False)):
-        xy = np.stack([b * np.cos(psi), b * np.sin(psi)], 1)
-        r = B.trace_points(st, cam, B.Emission(), it, xy)
-        wrong += int(np.sum((np.asarray(r["status"]) == 1) != captured))
+        xy = np.tile(np.stack([b * np.cos(psi), b * np.sin(psi)], 1), (28, 1))
+        status = np.asarray(B.trace_points(st, cam, B.Emission(), it, xy)["status"])[:400]
+        wrong += int(np.sum((status == 1) != captured))
     assert wrong <= 40
