@@ -406,13 +406,50 @@ struct bh_plan_s {
 
 namespace {
 
-// Tolerances at which the image path's FP64-accuracy rays run in split
-// arithmetic (step_split.cuh): its rounding, a few 2^-47 of the terms of a
-// step, is then four orders of magnitude below the truncation the tolerances
-// admit, and the image planes are floats.  Tighter tolerances keep the FP64
-// kernel, and so do FP64 volumetric images (their FP64 source g^3 j is most of
-// a step) and the records of bh_trace_points, which are doubles.
-bool split_allowed(double rtol, double atol) { return rtol >= 1e-10 && atol >= 1e-12; }
+// Images whose FP64-accuracy rays run in split arithmetic (step_split.cuh):
+// its rounding, a few 2^-47 of the terms of a step, has to stay well below the
+// truncation that the tolerances admit, and the image planes are floats.  All
+// others keep the FP64 kernel, as do FP64 volumetric images (their FP64 source
+// g^3 j is most of a step) and the records of bh_trace_points, which are
+// doubles.
+//   - Tolerances: rtol >= 1e-10 and atol >= 1e-12, four orders of magnitude
+//     above the rounding.
+//   - Cancellation: the right-hand side divides by Delta, which loses R^2 /
+//     Delta of its digits near the horizon (most at R_cap, where the domain
+//     ends), and by sin(theta), of which theta near pi leaves pi / sin(theta_o)
+//     for rays along the axis.  2^-46 of either has to be below rtol / 8: at
+//     rtol 1e-10 and the default R_cap = 1.01 R_+ up to chi = 0.998, with a
+//     constraint drift 1 % off the FP64 kernel's; at R_cap = 1.0001 R_+ it was
+//     1.7 times that, with 4 % more steps.
+//   - Range: constants that are ordinary floats with room for their squares (R
+//     up to ten times R_esc), and an emissivity exponent that stays in the
+//     floats: an overflow there is a NaN, where FP64 has a value.  e^x is 0
+//     below x = -87, at most 2^10 e^-87 = 2e-35 of intensity.
+bool split_allowed(const ImgParams& ip) {
+  if (!(ip.rtol >= 1e-10 && ip.rtol <= 1.0 && ip.atol >= 1e-12 && ip.atol <= 1e12)) return false;
+  double H, dH;
+  host_lapse(HostMetric{ip.metric, ip.chi, ip.lamE, ip.eta, ip.lamc}, ip.R_cap, H, dH);
+  const double R2 = ip.R_cap * ip.R_cap, D = R2 * H + ip.chi * ip.chi;
+  const double loss = std::fmax(R2 / D, kPi / ip.sin_o);
+  if (!(D > 0.0 && std::ldexp(loss, -46) <= 0.125 * ip.rtol)) return false;
+  auto within = [](double x, double lo, double hi) { return std::fabs(x) >= lo && std::fabs(x) <= hi; };
+  const double big = std::ldexp(1.0, 40);
+  if (!within(ip.R_esc, 0.0, big) || !within(ip.chi, 0.0, big)) return false;
+  if (ip.metric == BH_EINASTO && !within(ip.lamE, 1.0 / big, big)) return false;
+  if (ip.metric == BH_CNFW &&
+      !(within(ip.lamc, 1.0 / big, big) && within(ip.eta * ip.lamc, 0.0, big)))
+    return false;
+  const double rate = 4096.0;
+  if (!within(ip.R_in, 0.0, big) || !within(ip.R_out, 0.0, big) ||
+      !within(ip.isig_in, 0.0, rate) || !within(ip.isig_out, 0.0, rate) ||
+      !within(ip.iR_s, 0.0, rate) || !within(ip.p, 0.0, rate) ||
+      !(ip.j0 == 0.0 || within(ip.j0, std::ldexp(1.0, -64), 1024.0)))
+    return false;
+  // the largest exponent of (R / R_in)^-p e^-(R - R_in)/R_s on [R_cap, R_esc]
+  const double up = ip.p * std::log(ip.R_in / (ip.p > 0.0 ? ip.R_cap : ip.R_esc)) +
+                    std::fmax(0.0, (ip.R_in - ip.R_cap) * ip.iR_s);
+  return up <= 64.0;
+}
 
 int count_launches(const bh_plan_s& p) {
   const int passes = p.precision == 1 ? 3 : 1;
@@ -478,7 +515,7 @@ bh_status plan_build(int32_t n, const bh_spacetime* st, const bh_camera* cam,
   const int sms = num_sms();
   const int threads = 128;
   p.split = !(p.precision == 0 && p.any_vol);
-  for (int i = 0; i < n; ++i) p.split = p.split && split_allowed(integ[i].rtol, integ[i].atol);
+  for (int i = 0; i < n; ++i) p.split = p.split && split_allowed(p.ip[i]);
   p.shape.threads = threads;
   p.shape.blocks = sms * (p.precision == 0 ? blocks64(p, threads, 0)
                                            : trace_default_blocks_per_sm(1, threads));
@@ -869,7 +906,7 @@ bh_status bh_shadow_boundary(const bh_spacetime* st, const bh_camera* cam,
   // transition by that much of the truncation error.  Ends of 1e-9 wide brackets
   // re-traced by the FP64 kernel: of 400 a case, 0 disagreed at rtol 1e-10, 0 or
   // 1 at 1e-8, up to 5 at 1e-6, 170 at 1e-4
-  const bool split = split_allowed(integ->rtol, integ->atol) && integ->rtol <= 1e-8 &&
+  const bool split = split_allowed(ip) && integ->rtol <= 1e-8 &&
                      b_tol >= 1e-11;
   const int64_t resident = shadow_resident_threads(split);
   int G = 1;
