@@ -463,13 +463,18 @@ bh_status bh_visibility_curves(const float* I, const bh_camera* cam, int32_t n_q
  * decisions frozen (accepted step sizes, refinement pattern, trusted
  * crossings, termination step); R_in = r_ISCO or R_+ + dR_in is
  * differentiated implicitly; the capture radius is held fixed.
- * The forward pass runs in FP64 whatever integ->precision says.  Each ray
- * is replayed with a checkpoint every 64 accepted steps into a per-thread
- * slab sized from the forward image's longest ray (longer rays: fewer
- * threads share the workspace's checkpoint region); BH_ERR_WORKSPACE only
- * if one block of 128 such slabs does not fit there (on a 152-SM GPU, a
- * longest ray of more than about 1.2 million steps, above the default step
- * limit) or a ray has more than 32 trusted crossings.
+ * The forward image is that of precision 0; the rays are replayed in FP64.
+ * Kerr and Einasto images keep the replayed trajectories, 40 B a step, in what
+ * the workspace has beyond the image's own part, in several portions if they do
+ * not fit: bh_backward_workspace_size, enough for every metric, suits images up
+ * to about 90^2, and 45 KB a pixel more (up to 3 GB) makes larger ones three to
+ * four times faster; what the workspace cannot hold well, and cored-NFW images,
+ * replay each ray with a checkpoint every 64 accepted steps in a per-thread slab
+ * sized from the forward image's longest ray (longer rays: fewer threads share
+ * the checkpoint region).  BH_ERR_WORKSPACE only if one block of 128 such slabs
+ * does not fit there (on a 152-SM GPU, a longest ray of more than about 1.2
+ * million steps, above the default step limit) or a ray has more than 32 trusted
+ * crossings.
  * dL_dI (device float [ny][nx]), dL_ddiag (host, 11) and uv8 (host, 8x2
  * cycles/M) may be NULL; diag11 (host) receives D; image_out (device float
  * [ny][nx]) the forward intensity.  Synchronous: returns when grad10 is

@@ -683,6 +683,7 @@ def visibility_curves(I: torch.Tensor, cam: Camera, q, n_phi: int = 256, mode: i
 
 
 GRAD_NAMES = ["chi", "incl", "halo1", "halo2", "j0", "p", "R_s", "sigma_in", "sigma_out", "R_out"]
+_CHUNK_BYTES = 2800  # of a trajectory chunk with its share of the ray records
 LOSS_DIAG_NAMES = ["C", "A_LR", "rho_peak"] + [f"vis{k}" for k in range(8)]
 
 
@@ -697,7 +698,12 @@ def trace_backward(st: Spacetime, cam: Camera, em: Emission, integ: Integrator,
     nb = C.c_size_t(0)
     _check(lib().bh_backward_workspace_size(C.byref(cam._c()), C.byref(nb)),
            "bh_backward_workspace_size")
-    ws = _aligned_workspace(nb.value, device)
+    nbytes = nb.value
+    if st.metric != CNFW:
+        # room for the rays' trajectories (bh_trace_backward): 16 chunks of 64
+        # steps a pixel, up to 2^20 chunks
+        nbytes += _CHUNK_BYTES * min(16 * cam.nx * cam.ny, 1 << 20)
+    ws = _aligned_workspace(nbytes, device)
     grad = np.zeros(10)
     diag = np.zeros(11)
     img = torch.empty(cam.ny, cam.nx, dtype=torch.float32, device=device)

@@ -1154,14 +1154,11 @@ constexpr int kAdjBlocksPerSM = 2;
 // steps = 4096 accepted steps per ray); rays of the forward image that took
 // more steps get larger slabs and the adjoint runs on fewer threads
 constexpr int kAdjMaxCkpt = 64;
-// Room of one forward / reverse pair of adjoint_warp.cu (Kerr, Einasto):
-// trajectory chunks of kAdjChunk steps (40 B a step) and a ray record per four
-// chunks; an image that needs more takes several pairs.  The forward replay runs
-// on at most as many threads as the pool holds longest rays, so a pool that is
-// small against the image leaves SMs idle: 16 chunks a pixel, 0.67 to 2.7 GB.
-// Gradients of 256^2 and 448^2 Kerr images, one refinement level: adjoint.cu
-// 1,241 and 2,377 ms, 0.67 GB 1,252 and 2,778, 2.7 GB 295 and 1,089.
-constexpr int64_t kAdjMinChunks = 1 << 18;
+// Room of one forward / reverse pair of adjoint_warp.cu (Kerr, Einasto), in
+// what the caller's workspace has for the ray adjoint, which need not be more
+// than adjoint.cu's checkpoints: trajectory chunks of kAdjChunk steps (40 B a
+// step) and a ray record per four chunks, 2.8 KB a chunk; an image that needs
+// more takes several pairs.
 constexpr int64_t kAdjMaxChunks = 1 << 20;
 
 // Lapse H(R) for any scalar type: Kerr, Eq. (9) with halo1 = lambda_E,
@@ -1254,9 +1251,14 @@ AdjImg adjoint_constants(const bh_spacetime& s, const bh_camera& c, const bh_emi
 
 struct BwdLayout {
   Layout fwd;
-  size_t I, nc, st, G, mom, lr, hs, hc, uv, V, grad, head, status, ctl, ckpt, prev, ray, total;
+  size_t I, nc, st, G, mom, lr, hs, hc, uv, V, grad, head, status, room, total;
   int nbins, threads;
-  int64_t chunks, rays;  // of the trajectory pool, and its ray records
+};
+
+// The trajectory pool of adjoint_warp.cu, from `room` to the workspace's end.
+struct AdjRoom {
+  size_t ctl, pool, prev, ray;
+  int64_t chunks, rays;
 };
 
 bool bwd_layout(const bh_camera& c, BwdLayout& B) {
@@ -1289,16 +1291,23 @@ bool bwd_layout(const bh_camera& c, BwdLayout& B) {
   B.grad = take(sizeof(double) * 10);
   B.head = take(sizeof(unsigned long long));
   B.status = take(sizeof(int));
-  B.ctl = take(sizeof(AdjCtl));
-  // the checkpoints of adjoint.cu or the trajectory pool of adjoint_warp.cu
-  B.chunks = std::min(std::max(16 * npix, kAdjMinChunks), kAdjMaxChunks);
-  B.rays = B.chunks / 4;
-  B.ckpt = take(std::max(sizeof(Ckpt) * (size_t)B.threads * kAdjMaxCkpt,
-                         sizeof(double) * 5 * kAdjChunk * (size_t)B.chunks));
-  B.prev = take(sizeof(int32_t) * (size_t)B.chunks);
-  B.ray = take(sizeof(AdjRay) * (size_t)B.rays);
+  // the checkpoints of adjoint.cu, or the pool of adjoint_warp.cu
+  B.room = take(sizeof(Ckpt) * (size_t)B.threads * kAdjMaxCkpt);
   B.total = o;
   return true;
+}
+
+AdjRoom adj_room(const BwdLayout& B, size_t ws_bytes) {
+  AdjRoom r;
+  const size_t chunk = sizeof(double) * 5 * kAdjChunk + sizeof(int32_t) + sizeof(AdjRay) / 4;
+  const size_t have = ws_bytes - B.room;  // at least the checkpoints' size
+  r.chunks = std::min<int64_t>((int64_t)((have - 4 * 256) / chunk), kAdjMaxChunks) / 4 * 4;
+  r.rays = r.chunks / 4;
+  r.ctl = B.room;
+  r.pool = r.ctl + align256(sizeof(AdjCtl));
+  r.prev = r.pool + align256(sizeof(double) * 5 * kAdjChunk * (size_t)r.chunks);
+  r.ray = r.prev + align256(sizeof(int32_t) * (size_t)r.chunks);
+  return r;
 }
 
 }  // namespace
@@ -1459,77 +1468,86 @@ bh_status bh_trace_backward(const bh_spacetime* st, const bh_camera* cam, const 
   J.Gpix = A.G;
   J.base_child = ra.base_child;
   for (int l = 1; l <= kMaxLevels; ++l) J.lv[l] = ra.lv[l];
-  J.ckpt = reinterpret_cast<Ckpt*>(ws + BL.ckpt);
+  J.ckpt = reinterpret_cast<Ckpt*>(ws + BL.room);
   J.grad = reinterpret_cast<double*>(ws + BL.grad);
   J.head = reinterpret_cast<unsigned long long*>(ws + BL.head);
   J.status = reinterpret_cast<int*>(ws + BL.status);
   // room per ray from the forward image's longest ray: its attempted steps
-  // bound the accepted steps of the replay (the image's split steps can differ
-  // from the replay's by a few, hence the eighth more).  adjoint.cu: the
-  // workspace's checkpoint region is divided among as many threads as it can
-  // hold slabs of that many checkpoints, up to the default grid
+  // bound the accepted steps of the replay, an eighth more because the image's
+  // split steps can differ from the replay's
   unsigned long long longest = 0;
   if (cudaMemcpyAsync(&longest, &ra.hdr->max_ray_steps, sizeof(longest), cudaMemcpyDeviceToHost,
                       cs) != cudaSuccess ||
       cudaStreamSynchronize(cs) != cudaSuccess)
     return BH_ERR_CUDA;
-  const unsigned long long spare = longest / 8;
-  if (cudaMemsetAsync(ws + BL.grad, 0, BL.ctl - BL.grad, cs) != cudaSuccess) return BH_ERR_CUDA;
-  if (st->metric != BH_CNFW) {
-    AdjWarpArgs K;
-    std::memset(&K, 0, sizeof(K));
-    K.hdr = J.hdr;
-    K.ip = J.ip;
-    K.aj = J.aj;
-    K.levels = J.levels;
-    K.npix = npix;
-    K.Gpix = J.Gpix;
-    K.base_child = J.base_child;
-    for (int l = 1; l <= kMaxLevels; ++l) K.lv[l] = J.lv[l];
-    K.grad = J.grad;
-    K.head = J.head;
-    K.status = J.status;
-    K.ctl = reinterpret_cast<AdjCtl*>(ws + BL.ctl);
-    K.pool = reinterpret_cast<double*>(ws + BL.ckpt);
-    K.prev = reinterpret_cast<int32_t*>(ws + BL.prev);
-    K.chunks = BL.chunks;
-    K.ray = reinterpret_cast<AdjRay*>(ws + BL.ray);
-    K.max_rays = BL.rays;
-    K.per_ray = (int)std::min<unsigned long long>((longest + spare) / kAdjChunk + 2,
-                                                  (unsigned long long)BL.chunks + 1);
-    const int64_t most = std::min<int64_t>(BL.threads, BL.chunks / K.per_ray);
-    if (most < 1) return BH_ERR_WORKSPACE;
-    const int fthreads = (int)std::min<int64_t>(most, kAdjThreads);
-    for (bool more = true; more;) {
-      AdjCtl ctl;
-      if (cudaMemsetAsync(K.ctl, 0, sizeof(AdjCtl), cs) != cudaSuccess ||
-          launch_adj_forward(K, (int)(most / fthreads), fthreads, cs) != cudaSuccess ||
-          launch_adj_reverse(K, cs) != cudaSuccess ||
-          cudaMemcpyAsync(&ctl, K.ctl, sizeof(ctl), cudaMemcpyDeviceToHost, cs) != cudaSuccess ||
-          cudaStreamSynchronize(cs) != cudaSuccess)
-        return BH_ERR_CUDA;
-      // a pair that neither ended the list nor took a ray could not go on
-      more = ctl.done == 0 && ctl.rays > 0;
+  const AdjRoom W = adj_room(BL, workspace_bytes);
+  const int64_t most_steps = (int64_t)longest;
+  int dstat = 0;
+  {
+    const int64_t n = most_steps + most_steps / 8;
+    if (cudaMemsetAsync(ws + BL.grad, 0, BL.room - BL.grad, cs) != cudaSuccess) return BH_ERR_CUDA;
+    // adjoint_warp.cu for Kerr and Einasto while its forward replay finds room
+    // for a quarter of the threads that the image could use: it runs on at most
+    // as many as the pool holds longest rays.  Kerr images with one refinement
+    // level, adjoint.cu against pools of 2^18 and 2^20 chunks: 256^2 1,241,
+    // 1,252 and 295 ms, 448^2 (longest ray 1,866 steps) 2,377, 2,778 and 1,089
+    const int64_t per = n / kAdjChunk + 2;
+    const int64_t most = std::min<int64_t>(BL.threads, W.chunks / per);
+    if (st->metric != BH_CNFW && 4 * most >= std::min<int64_t>(BL.threads, npix)) {
+      AdjWarpArgs K;
+      std::memset(&K, 0, sizeof(K));
+      K.hdr = J.hdr;
+      K.ip = J.ip;
+      K.aj = J.aj;
+      K.levels = J.levels;
+      K.npix = npix;
+      K.Gpix = J.Gpix;
+      K.base_child = J.base_child;
+      for (int l = 1; l <= kMaxLevels; ++l) K.lv[l] = J.lv[l];
+      K.grad = J.grad;
+      K.head = J.head;
+      K.status = J.status;
+      K.ctl = reinterpret_cast<AdjCtl*>(ws + W.ctl);
+      K.pool = reinterpret_cast<double*>(ws + W.pool);
+      K.prev = reinterpret_cast<int32_t*>(ws + W.prev);
+      K.chunks = W.chunks;
+      K.ray = reinterpret_cast<AdjRay*>(ws + W.ray);
+      K.max_rays = W.rays;
+      K.per_ray = (int)per;
+      const int fthreads = (int)std::min<int64_t>(most, kAdjThreads);
+      for (bool more = true; more;) {
+        AdjCtl ctl;
+        if (cudaMemsetAsync(K.ctl, 0, sizeof(AdjCtl), cs) != cudaSuccess ||
+            launch_adj_forward(K, (int)(most / fthreads), fthreads, cs) != cudaSuccess ||
+            launch_adj_reverse(K, cs) != cudaSuccess ||
+            cudaMemcpyAsync(&ctl, K.ctl, sizeof(ctl), cudaMemcpyDeviceToHost, cs) != cudaSuccess ||
+            cudaStreamSynchronize(cs) != cudaSuccess)
+          return BH_ERR_CUDA;
+        more = ctl.done == 0;
+        if (more && ctl.rays == 0) return BH_ERR_WORKSPACE;  // a pair that took no ray
+      }
+    } else {
+      // the checkpoint region is divided among as many threads as it can hold
+      // slabs of the longest ray's checkpoints, up to the default grid
+      const int64_t room = (int64_t)BL.threads * kAdjMaxCkpt;
+      auto slabs = [&](int64_t steps) {
+        const int64_t c = std::max<int64_t>(kAdjMaxCkpt, steps / kCkptEvery + 2);
+        return std::min<int64_t>(BL.threads, room / c) / kAdjThreads * kAdjThreads;
+      };
+      int64_t threads = slabs(n);
+      if (threads < kAdjThreads) threads = slabs(most_steps);
+      if (threads < kAdjThreads) return BH_ERR_WORKSPACE;
+      J.max_ckpt = (int)std::min<int64_t>(room / threads, 1 << 30);
+      // one-warp blocks: a 48^2 gradient took 605, 513 and 502 ms with blocks of
+      // 128, 64 and 32 threads (an image's rays spread over more SMs)
+      if (launch_adjoint(J, (int)(threads / 32), 32, cs) != cudaSuccess) return BH_ERR_CUDA;
     }
-  } else {
-    const int64_t room = (int64_t)BL.threads * kAdjMaxCkpt;  // checkpoints in the region
-    int64_t threads = 0;
-    for (unsigned long long n = longest + spare; threads < kAdjThreads; n = longest) {
-      const int64_t per = std::max<int64_t>(kAdjMaxCkpt, (int64_t)(n / kCkptEvery) + 2);
-      threads = std::min<int64_t>(BL.threads, room / per) / kAdjThreads * kAdjThreads;
-      if (n == longest) break;
-    }
-    if (threads < kAdjThreads) return BH_ERR_WORKSPACE;
-    J.max_ckpt = (int)std::min<int64_t>(room / threads, 1 << 30);
-    // one-warp blocks: a 48^2 gradient took 605, 513 and 502 ms with blocks of
-    // 128, 64 and 32 threads (an image's rays spread over more SMs)
-    if (launch_adjoint(J, (int)(threads / 32), 32, cs) != cudaSuccess)
+    if (cudaMemcpyAsync(&dstat, J.status, sizeof(int), cudaMemcpyDeviceToHost, cs) != cudaSuccess ||
+        cudaStreamSynchronize(cs) != cudaSuccess)
       return BH_ERR_CUDA;
   }
-  int dstat = 0;
   if (cudaMemcpyAsync(grad10, J.grad, sizeof(double) * 10, cudaMemcpyDeviceToHost, cs) !=
-          cudaSuccess ||
-      cudaMemcpyAsync(&dstat, J.status, sizeof(int), cudaMemcpyDeviceToHost, cs) != cudaSuccess)
+      cudaSuccess)
     return BH_ERR_CUDA;
   if (image_out &&
       cudaMemcpyAsync(image_out, I, sizeof(float) * npix, cudaMemcpyDeviceToDevice, cs) !=
