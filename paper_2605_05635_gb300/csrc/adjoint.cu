@@ -315,11 +315,11 @@ __global__ void __launch_bounds__(128) adjoint_kernel(AdjArgs a) {
     double pdir[13];  // direct adjoint of the crossing terms (tangents of D13)
     for (int t = 0; t < 13; ++t) pdir[t] = 0.0;
     int nck = 0;
-    bool overflow = false;
+    int overflow = 0;
     while (true) {
       if (r.nacc % kCkptEvery == 0 && r.nacc / kCkptEvery == nck && !r.rejected) {
         if (nck >= a.max_ckpt) {
-          overflow = true;
+          overflow = kAdjNoRoom;
           break;
         }
         save_ckpt(r, ck[nck++]);
@@ -336,12 +336,12 @@ __global__ void __launch_bounds__(128) adjoint_kernel(AdjArgs a) {
           for (int t = 1; t < 13; ++t) pdir[t] += gI * Ic.d[t];
         }
         if (nx < kMaxCrossAdj) xr[nx++] = XRec{r.nacc - 1, sig, Rb};
-        else overflow = true;
+        else overflow = (int)BH_ERR_WORKSPACE;
       }
       if (term) break;
     }
     if (overflow) {
-      atomicCAS(a.status, 0, (int)BH_ERR_WORKSPACE);
+      atomicCAS(a.status, 0, overflow);
       continue;
     }
     if (nx == 0) continue;

@@ -9,6 +9,8 @@ namespace bhrt {
 
 constexpr int kCkptEvery = 64;
 constexpr int kMaxCrossAdj = 32;
+// device status of a ray that ran out of checkpoints or chunks (no bh_status)
+constexpr int kAdjNoRoom = -1;
 
 // Derivatives of per-image constants with respect to (chi, theta_o, halo1,
 // halo2), computed on the host.

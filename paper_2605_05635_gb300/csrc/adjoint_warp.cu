@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(128) adj_forward_kernel(AdjWarpArgs a) {
     AdjRay& rec = a.ray[atomicAdd(&a.ctl->rays, 1ull)];
     int nx = 0, used = 0;
     int32_t chunk = -1;
-    bool overflow = false;
+    int overflow = 0;
     while (true) {
       const int n = r.nacc;
       const double y0 = r.y[1], y1 = r.y[2], y2 = r.y[4], y3 = r.y[5], h0 = r.h;
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(128) adj_forward_kernel(AdjWarpArgs a) {
         const int i = n % kAdjChunk;
         if (i == 0) {
           if (used >= a.per_ray) {
-            overflow = true;
+            overflow = kAdjNoRoom;
             break;
           }
           const int32_t c = (int32_t)atomicAdd(&a.ctl->used, 1ull);  // reserved: there is one
@@ -265,12 +265,12 @@ __global__ void __launch_bounds__(128) adj_forward_kernel(AdjWarpArgs a) {
           for (int t = 1; t < 13; ++t) pdir[t] += gI * Ic.d[t];
         }
         if (nx < kMaxCrossAdj) rec.x[nx++] = XRec{r.nacc - 1, sig, Rb};
-        else overflow = true;
+        else overflow = (int)BH_ERR_WORKSPACE;
       }
       if (term) break;
     }
     if (overflow) {
-      atomicCAS(a.status, 0, (int)BH_ERR_WORKSPACE);
+      atomicCAS(a.status, 0, overflow);
       nx = 0;
     }
     rec.nx = nx;

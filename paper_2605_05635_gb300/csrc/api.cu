@@ -1474,7 +1474,9 @@ bh_status bh_trace_backward(const bh_spacetime* st, const bh_camera* cam, const 
   J.status = reinterpret_cast<int*>(ws + BL.status);
   // room per ray from the forward image's longest ray: its attempted steps
   // bound the accepted steps of the replay, an eighth more because the image's
-  // split steps can differ from the replay's
+  // split steps can differ from the replay's; a ray that needs more yet (one
+  // next to the critical curve that stays there longer in the replay) has the
+  // whole adjoint run again with twice the room
   unsigned long long longest = 0;
   if (cudaMemcpyAsync(&longest, &ra.hdr->max_ray_steps, sizeof(longest), cudaMemcpyDeviceToHost,
                       cs) != cudaSuccess ||
@@ -1483,8 +1485,7 @@ bh_status bh_trace_backward(const bh_spacetime* st, const bh_camera* cam, const 
   const AdjRoom W = adj_room(BL, workspace_bytes);
   const int64_t most_steps = (int64_t)longest;
   int dstat = 0;
-  {
-    const int64_t n = most_steps + most_steps / 8;
+  for (int64_t n = most_steps + most_steps / 8;; n *= 2) {
     if (cudaMemsetAsync(ws + BL.grad, 0, BL.room - BL.grad, cs) != cudaSuccess) return BH_ERR_CUDA;
     // adjoint_warp.cu for Kerr and Einasto while its forward replay finds room
     // for a quarter of the threads that the image could use: it runs on at most
@@ -1535,7 +1536,7 @@ bh_status bh_trace_backward(const bh_spacetime* st, const bh_camera* cam, const 
         return std::min<int64_t>(BL.threads, room / c) / kAdjThreads * kAdjThreads;
       };
       int64_t threads = slabs(n);
-      if (threads < kAdjThreads) threads = slabs(most_steps);
+      if (threads < kAdjThreads && n == most_steps + most_steps / 8) threads = slabs(most_steps);
       if (threads < kAdjThreads) return BH_ERR_WORKSPACE;
       J.max_ckpt = (int)std::min<int64_t>(room / threads, 1 << 30);
       // one-warp blocks: a 48^2 gradient took 605, 513 and 502 ms with blocks of
@@ -1545,6 +1546,7 @@ bh_status bh_trace_backward(const bh_spacetime* st, const bh_camera* cam, const 
     if (cudaMemcpyAsync(&dstat, J.status, sizeof(int), cudaMemcpyDeviceToHost, cs) != cudaSuccess ||
         cudaStreamSynchronize(cs) != cudaSuccess)
       return BH_ERR_CUDA;
+    if (dstat != kAdjNoRoom) break;
   }
   if (cudaMemcpyAsync(grad10, J.grad, sizeof(double) * 10, cudaMemcpyDeviceToHost, cs) !=
       cudaSuccess)
