@@ -96,7 +96,7 @@ def test_critical_rays_on_both_kernels(B, tol, steps):
     """A screen straddling the critical curve.  At rtol 1e-10 the forward image's split
     rays and the FP64 replay part next to it; at 1e-15 the longest ray takes more
     than the 64 checkpoints of 64 steps that a thread has by default."""
-    ext = (4.3, 4.5, -0.1, 0.1)
+    ext = (3.9, 4.9, -0.5, 0.5)
     kw = dict(chi=0.9, incl=80.0, ext=ext, rtol=tol, atol=1e-2 * tol)
     kerr, nfw = _item(B, 0, 32, 3, **kw), _item(B, 2, 32, 3, eta=0.0, **kw)
     p = B.Plan([kerr])
