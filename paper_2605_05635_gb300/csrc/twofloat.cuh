@@ -128,12 +128,6 @@ BH_HD F2 mulf_raw(float x, F2 y) {
 }
 // c + x y
 BH_HD F2 fma2(F2 x, F2 y, F2 c) { return add(c, mul_raw(x, y)); }
-// the running sum s + x y, left unnormalised (s.l collects the small terms)
-BH_HD F2 acc2(F2 x, F2 y, F2 s) {
-  const F2 p = mul_raw(x, y);
-  const F2 t = two_sum(s.h, p.h);
-  return mk2(t.h, f_add(s.l, f_add(t.l, p.l)));
-}
 // a Horner step c + z t where |c| >= |z t|, left unnormalised
 BH_HD F2 horner2(F2 z, F2 t, F2 c) {
   const F2 p = mul_raw(z, t);
