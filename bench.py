@@ -956,7 +956,7 @@ def run_profile_case(args):
     128^2 over [-10, 10]^2, no refinement), ``sweep512`` (the first image of
     the 512^2 sweep, with refinement), ``sweep512l0`` (the same image without
     refinement), ``shadow512`` (the Fig. 5 cored-NFW shadow boundary along
-    512 directions to 1e-10, FP64), ``scan64k`` (65,536 spacetimes of the
+    512 directions to 1e-10), ``scan64k`` (65,536 spacetimes of the
     Figs. 3-4 grids with 16 angles).  Tracing cases use the chosen
     precision's integrator settings."""
     import torch

@@ -112,30 +112,44 @@ typedef struct {
                          no timelike orbit exists, and steps that may come
                          within 5 H of the plane advancing z by at most H/2.
                          I_n planes stay 0; H0 > 0 and h >= 0 required.
-                         The all-FP64 path evaluates the source g^3 j in
-                         FP64; the mixed path evaluates it in FP32 on every
-                         leg (the promoted FP64 steps keep an FP64
-                         geodesic).  Not differentiable by bh_trace_backward. */
+                         The FP64 path evaluates the source g^3 j and the
+                         geodesic in FP64; the mixed path evaluates the
+                         source in FP32 on every leg (the promoted steps
+                         keep a geodesic of FP64 accuracy).  Not
+                         differentiable by bh_trace_backward. */
   double j0, p, R_s;  /* normalisation, radial power, radial scale (Eq. 83) */
   double sigma_in, sigma_out, R_out; /* tapers, Eqs. (85)-(86)             */
   double dR_in;       /* used when r_in_mode == 1                           */
   double H0, h;       /* disk height H(rho) = H0 + h rho, Eq. (84)          */
 } bh_emission;
 
-/* Integrator (the paper names none; these are the build's readings). */
+/* Integrator (the paper names none; these are the build's readings).
+ *
+ * Steps of FP64 accuracy (precision 0 images, the mixed path's promoted rays,
+ * shadow boundaries) run in one of two arithmetics.  Thin-disk rays take split
+ * steps, sums of two or three floats (48 bits in a step, 72 in the state) on the
+ * FP32 pipes, where that cannot be told from FP64 in float planes: rtol >= 1e-10
+ * and atol >= 1e-12, a capture radius and an inclination at which the
+ * cancellation next to the horizon (R^2 / Delta at R_cap) and the axis (pi /
+ * sin theta_o) stays below 2^43 rtol, and constants of float range (esc_factor
+ * R_o and R_out up to 2^40, rates of the emissivity up to 2^12, |j0| 2^-64 to
+ * 2^10, or 0; intensities below about 1e-35 come out as 0).  All other rays, and
+ * the records of bh_trace_points, are FP64 throughout: an atol just below 1e-12
+ * asks for that.  The images of one call share the choice. */
 typedef struct {
-  int32_t precision;    /* 0: all-FP64; 1: mixed (FP32 bulk, FP64 promoted) */
+  int32_t precision;    /* 0: FP64 accuracy; 1: mixed (FP32 bulk, promoted
+                           rays of FP64 accuracy)                         */
   int32_t max_steps;    /* attempted steps per ray before status 2          */
   double rtol, atol;    /* Dormand-Prince 5(4) tolerances                   */
   double cap_factor;    /* capture when R < cap_factor * R_+ (Eq. 75)       */
   double esc_factor;    /* escape when R > esc_factor * R_o                 */
   double thetadot_min;  /* trusted crossing needs |dtheta/dlambda| >= this  */
   double dlambda_min;   /* and an affine gap >= this to the previous one    */
-  double promote_dr;    /* mixed: FP64 steps while R < R_+ + promote_dr     */
+  double promote_dr;    /* mixed: promoted while R < R_+ + promote_dr       */
   double time_budget_s; /* device time budget per call (s); 0 = none      */
   int32_t promote_order;/* mixed: rays reaching image order n >= this
-                           (n = N_cross - 1, Sec. 4.2) inside R = 5 take
-                           FP64 steps until outgoing beyond R = 5;
+                           (n = N_cross - 1, Sec. 4.2) inside R = 5 are
+                           promoted until outgoing beyond R = 5;
                            0..1000, 1000 = never                          */
   int32_t reserved;     /* must be 0                                        */
   double promote_turning; /* mixed: radial turning points of near-critical
@@ -143,15 +157,15 @@ typedef struct {
                            Hamiltonian (Eqs. 56-59), Rr(R) = P^2 - Delta K =
                            (Delta p_R)^2, P = (R^2 + chi^2) E - chi ell and K
                            the Carter-type constant p_th^2 + Q^2, a ray inside
-                           R = 5 takes FP64 steps once Rr < kappa P^2 and
+                           R = 5 is promoted once Rr < kappa P^2 and
                            Rr'^2 < 2 kappa Rr'' P^2 (Rr'' with Kerr's
                            Delta'' = 2): it is within kappa of a double root
                            of Rr, i.e. near the photon orbit, about to turn
                            or to plunge; it returns to FP32 once outgoing
                            beyond R = 5 or with Rr > 1.2 kappa P^2 (past the
                            root).  kappa = promote_turning in [0, 1];
-                           0 = off.  Every FP32 -> FP64 hand-off also puts
-                           p_th and p_R back on the ray's FP64 constants
+                           0 = off.  Every promotion also puts p_th and
+                           p_R back on the ray's FP64 constants
                            E, ell (Eq. 48) and K from the launch, with
                            the null condition (Eq. 54).                   */
 } bh_integrator;
@@ -178,8 +192,8 @@ typedef struct {
   int32_t* steps;         /* optional [2][ny*nx]: accepted and rejected
                              Dormand-Prince steps of the base ray (all
                              precisions together)                          */
-  uint8_t* promoted;      /* optional [ny*nx]: 1 if the base ray took FP64
-                             steps on the mixed path, else 0               */
+  uint8_t* promoted;      /* optional [ny*nx]: 1 if the base ray was
+                             promoted on the mixed path, else 0            */
 } bh_image_out;
 
 /* Per-ray record returned by bh_trace_points (device array of structs). */
@@ -225,8 +239,8 @@ bh_status bh_trace_batch(int32_t n, const bh_spacetime* st, const bh_camera* cam
 
 /* Traces single rays from explicit screen points xy[2*k], xy[2*k+1]
  * (device doubles) into records[k] (device).  Same physics as the image
- * path, no refinement; the mixed precision runs the image path's passes
- * (FP32, FP64 for promoted rays, FP32 after demotion).  Needs
+ * path, no refinement, steps of precision 0 and promoted rays in FP64; the mixed
+ * precision runs the image path's passes (FP32, promoted, FP32 after demotion).  Needs
  * bh_points_workspace_size(n) bytes (256-byte aligned). */
 bh_status bh_points_workspace_size(int64_t n, size_t* bytes);
 bh_status bh_trace_points(const bh_spacetime* st, const bh_camera* cam, const bh_emission* em,
@@ -248,7 +262,9 @@ bh_status bh_trace_points(const bh_spacetime* st, const bh_camera* cam, const bh
  * hole, 1 no horizon (|chi| > chi_e), 2 invalid parameters (unknown metric,
  * lambda_E <= 0, lambda_c <= 0, eta < 0 or a non-finite value; outputs 0).
  * stats (optional device int64[2], may be NULL) receives the lapse
- * evaluations H(R) of the horizon and of the stationary-limit searches.
+ * evaluations H(R) of the horizon (431 of them FP32 samples) and of the
+ * stationary-limit searches.  A spin equal to chi_e in its last bits may be
+ * flagged either way.
  * All arrays are device arrays; no workspace; asynchronous on stream. */
 bh_status bh_geometry_scan(int64_t n, const bh_spacetime* st, int32_t n_theta,
                            const double* theta, double* r_plus, double* chi_e, double* R_e,
@@ -267,14 +283,18 @@ bh_status bh_geometry_scan(int64_t n, const bh_spacetime* st, int32_t n_theta,
  * workspace status is then BH_ERR_TIMEOUT).  A bracket whose width can no
  * longer shrink in FP64 stops there.  If the fate is not monotone in b along
  * a direction, the transition nearest to b_lo among those the samples see
- * is returned.  Rays are traced by the FP64 integrator (integ->precision
- * must be 0) with the tolerances, step limit and thresholds of integ; the
+ * is returned.  Rays are traced with FP64 accuracy (integ->precision must
+ * be 0) and the tolerances, step limit and thresholds of integ: in split steps
+ * (see bh_integrator) where those apply, rtol <= 1e-8 and b_tol >= 1e-11, else in
+ * FP64; "captured" is the fate of the ray so traced.  The first samples lie
+ * around the critical impact parameter of the separated radial potential.  The
  * camera gives R_o and the inclination (its screen extent and pixel counts
  * are not used); emission plays no part.  Requires 0 <= b_lo < b_hi,
  * b_tol > 0, all finite (else BH_ERR_INVALID_ARG).  lanes: rays traced per
  * direction and round (1 = bisection, 2 .. 32 = (lanes + 1)-section; a power
  * of two), or 0 for the library's choice: the most lanes, up to 32, with
- * which all directions fit in half of the GPU's resident threads.  stats
+ * which all directions fit in 1.25 times (FP64 rays: half) of the GPU's resident
+ * threads.  stats
  * (optional device int64[3], may be NULL) receives the rays traced and their
  * accepted and rejected Dormand-Prince steps.  Needs
  * bh_shadow_workspace_size(n_psi) bytes of 256-byte aligned workspace. */
@@ -298,27 +318,28 @@ typedef struct bh_plan_s* bh_plan;
 typedef struct {
   int64_t cells[4];        /* cells per level (level 0 = n * nx * ny)         */
   int64_t rays[4];         /* rays integrated to termination per level        */
-  int64_t accepted_fp64;   /* accepted Dormand-Prince steps taken in FP64     */
-  int64_t rejected_fp64;   /* rejected FP64 trial steps                       */
+  int64_t accepted_fp64;   /* accepted steps of FP64 accuracy (split or FP64) */
+  int64_t rejected_fp64;   /* rejected trial steps of FP64 accuracy           */
   int64_t accepted_fp32;   /* mixed precision: accepted FP32 steps            */
   int64_t rejected_fp32;   /* mixed precision: rejected FP32 trial steps      */
-  int64_t promoted_rays;   /* mixed precision: rays handed to the FP64 pass   */
+  int64_t promoted_rays;   /* mixed precision: rays handed to the promoted pass */
   int64_t spill_full;      /* promotions refused because the queue was full   */
   int64_t max_ray_steps;   /* attempted steps of the longest ray              */
   double trace_ms[4];      /* per-level trace time (all passes) of the last
                               launch when timing is on, else -1               */
-  double fp32_ms, fp64_ms; /* trace kernel time by precision (timing on)      */
+  double fp32_ms, fp64_ms; /* trace kernel time, FP32 and FP64-accuracy passes
+                              (timing on)                                     */
   int32_t kernel_launches; /* kernels enqueued per launch                     */
   int32_t status;          /* device status word (bh_status)                  */
   int32_t trace_blocks, trace_threads; /* trace launch shape in use           */
-  /* Persistent-queue timeline per trace pass (0 main, 1 FP64 promoted,
+  /* Persistent-queue timeline per trace pass (0 main, 1 promoted,
    * 2 FP32 demoted) and level, from the device clock: bulk = first warp
    * start to the first warp finding the queue empty; tail = from then to
    * the last warp exit (warps running with idle lanes).  -1 if not run. */
   double bulk_ms[3][4];
   double tail_ms[3][4];
   /* Mean fraction of the 32 lanes holding a ray over the stepping-loop
-   * iterations of the FP32 and FP64 trace kernels (-1 if not run). */
+   * iterations of the FP32 and the FP64-accuracy trace kernels (-1 if not run). */
   double lane_util_fp32, lane_util_fp64;
 } bh_run_stats;
 
@@ -332,8 +353,8 @@ bh_status bh_plan_launch(bh_plan plan, int32_t use_graph, void* stream);
 /* Records CUDA events around each trace launch (disables graph replay). */
 bh_status bh_plan_set_timing(bh_plan plan, int32_t enable);
 /* Fixes the launch shape of a persistent trace kernel of the plan: which = 0
- * the main kernel (FP64, or the FP32 bulk of the mixed path), 1 the FP64
- * promoted pass; blocks >= 1, threads 64 or 128 (a multiple of 32),
+ * the main kernel of the mixed path (its FP32 bulk), 1 the kernel of the
+ * FP64-accuracy rays (all of precision 0, or the promoted pass); blocks >= 1, threads 64 or 128 (a multiple of 32),
  * variant 0 or 1 (the kernel build, as in bh_tune_report).  A grid smaller
  * than the GPU's resident capacity leaves room for other work, e.g. a second
  * plan on another stream.  Any captured graph is discarded. */
@@ -351,11 +372,12 @@ bh_status bh_plan_destroy(bh_plan plan);
  * results. */
 typedef struct {
   int32_t candidates;      /* shapes tried                                    */
-  int32_t blocks[2];       /* chosen grid: [0] main trace kernel, [1] FP64 pass */
+  int32_t blocks[2];       /* chosen grid: [0] main trace kernel, [1] promoted pass */
   int32_t threads[2];      /* chosen block size                               */
   double best_ms[2];       /* trace time of the whole launch with the choice  */
-  int32_t variant[2];      /* kernel build chosen: 0 registers unbounded,
-                              1 capped (FP64: 3 blocks of 128 per SM; mixed: 4) */
+  int32_t variant[2];      /* kernel build chosen: 0 registers unbounded (split:
+                              3 blocks of 128 per SM), 1 capped (FP64: 3; mixed
+                              and split: 4)                                   */
 } bh_tune_report;
 bh_status bh_plan_autotune(bh_plan plan, void* stream, bh_tune_report* report);
 
@@ -370,7 +392,9 @@ bh_status bh_plan_autotune(bh_plan plan, void* stream, bh_tune_report* report);
  * Integrals are pixel sums times dX dY at pixel centres; the left/right split
  * uses strict inequalities; the radial profile bins rho_0 (Eq. 105) with
  * width dX from 0, takes the mean per non-empty bin, resolves argmax ties to
- * the smaller radius and reports the bin centre.  All accumulation is FP64.
+ * the smaller radius and reports the bin centre.  Accumulation is FP64, the
+ * profile's bins exact integer sums where those hold at least as much (not with
+ * infinities, NaN or large negative values: then FP64 too).
  * Needs bh_diagnostics_workspace_size bytes of 256-byte aligned workspace. */
 bh_status bh_diagnostics_workspace_size(const bh_camera* cam, size_t* bytes);
 bh_status bh_diagnostics(const float* I, const bh_camera* cam, double theta_g, double* out12,

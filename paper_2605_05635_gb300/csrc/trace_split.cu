@@ -1,7 +1,7 @@
 // trace_split.cu -- persistent per-ray kernel of the image path in split
 // arithmetic (step_split.cuh): the rays of an FP64 image, and the promoted
 // pass of the mixed path.  Method, scheduling, events and hand-offs as in
-// trace.cu; the launch and the crossing events are FP64.
+// trace.cu; the launch is FP64, the crossing events two-float too.
 //
 // The FP64 kernel it replaces there is bound by the FP64 pipe (about 1,100
 // FP64 instructions per warp and step at 16 cycles each).  This one is bound
@@ -14,7 +14,7 @@
 //     their own (promote_kernel) in which every lane has a ray, and hand-off
 //     records carry float pairs, so starting or leaving the pass converts
 //     nothing;
-//   - crossings are parked as floats and evaluated in FP64 for several lanes
+//   - crossings are parked as floats and evaluated (cross_split) for several lanes
 //     together; a ray that ends with a parked crossing waits for the others.
 // Measured (GB300): the promoted passes of three mixed 512^2 images (one a
 // metric, 3 refinement levels) 676 -> 100 ms, a cored-NFW FP64 image of 96 x 75
