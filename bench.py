@@ -46,8 +46,7 @@ KEYS_CAP = 1 << 23                 # refinement-pattern keys kept per image
 # current kernels (dram__bytes_read.sum + dram__bytes_write.sum over the
 # kernel's launches of one plan launch); to be retaken whenever a trace kernel
 # changes.  Not measured for the volumetric layer, which reports null.
-# Not measured for trace_split_kernel either.
-TRAFFIC_PER_STEP = {"trace_mixed_kernel": 2.15e9}
+TRAFFIC_PER_STEP = {"trace_mixed_kernel": 2.15e9, "trace_split_kernel": 2.26e9}
 FP32_PEAK_FLOPS = 152 * 128 * 2 * 2.07e9   # 152 SMs x 128 FP32 lanes x FMA x 2.07 GHz
 # The FP64 images' rays and the mixed path's promoted rays take their steps in
 # split (two-float) arithmetic on the FP32 pipes, several FP32 operations for

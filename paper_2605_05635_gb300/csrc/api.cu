@@ -1540,7 +1540,8 @@ bh_status bh_trace_backward(const bh_spacetime* st, const bh_camera* cam, const 
       if (threads < kAdjThreads) return BH_ERR_WORKSPACE;
       J.max_ckpt = (int)std::min<int64_t>(room / threads, 1 << 30);
       // one-warp blocks: a 48^2 gradient took 605, 513 and 502 ms with blocks of
-      // 128, 64 and 32 threads (an image's rays spread over more SMs)
+      // 128, 64 and 32 threads (an image's rays spread over more SMs; runs of one
+      // shape differ by up to a tenth)
       if (launch_adjoint(J, (int)(threads / 32), 32, cs) != cudaSuccess) return BH_ERR_CUDA;
     }
     if (cudaMemcpyAsync(&dstat, J.status, sizeof(int), cudaMemcpyDeviceToHost, cs) != cudaSuccess ||
